@@ -433,8 +433,10 @@ tn_status tn_ite_run(tn_lattice *lat, const tn_ite_params *params, double *energ
  *          tensor cores (else FP32 SIMT); FP64 products of at least 64 x 64
  *          outputs and 128 terms, and FP32 ones from 2^26 multiply-adds, as
  *          exact BF16 digit products on the tensor cores, at the accuracy of
- *          FP64 and FP32 (else the FP64 and FP32 pipes).  Their digit planes
- *          take 14 and 6 bytes per operand entry; where only that exceeds the
+ *          FP64 and FP32 (else the FP64 and FP32 pipes; outputs whose terms
+ *          lie far below their row's and column's largest entries are left to
+ *          these pipes in either case).  Their digit planes
+ *          take 15 and 7 bytes per operand entry; where only that exceeds the
  *          budget left, every call falls back to the products without them
  *   bit 4  BF16x3 / BF16x6: smaller products on the tensor cores too
  *   bit 5  energies and correlators: the recompute form -- the corner chains

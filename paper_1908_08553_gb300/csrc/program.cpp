@@ -273,15 +273,16 @@ public:
         const int64_t Rp = (R + rpad - 1) / rpad * rpad, Kp = (Kd + kpad - 1) / kpad * kpad;
         int level = std::max(level_of(src), gfloor_) + 1;
         if (slices) level = std::max({level, level_of(k_self) + 1, level_of(k_other) + 1});
-        // BF16 planes (and a row exponent per digit row) in units of the arena's type
-        const int out = tensor(((int64_t)np * Rp * Kp * 2 + (slices ? Rp * 4 : 0)) / pg_.esize, level);
+        // BF16 planes (and a row exponent and the magnitudes per digit row) in units of the arena's type
+        const int out = tensor(((int64_t)np * Rp * Kp * 2 + (slices ? Rp * 4 + slice_mag_bytes(Rp, Kd) : 0)) / pg_.esize,
+                               level);
         Op op;
         op.kind = OP_TC_SPLIT;
         op.level = level;
         op.A = src; op.out = out;
         op.gm = R; op.gk = Kd; op.sam = sr; op.sak = sk;
         op.Rp = Rp; op.Kp = Kp; op.nsplit = np;
-        op.bytes = (double)R * Kd * pg_.esize + (double)np * Rp * Kp * 2;
+        op.bytes = (double)R * Kd * pg_.esize + (double)np * Rp * Kp * 2 + (slices ? (double)slice_mag_bytes(Rp, Kd) : 0.0);
         op.B = k_self; op.C = k_other; op.transE = first; op.slices = slices;
         use(src, level);
         if (slices) { use(k_self, level); use(k_other, level); }
@@ -311,6 +312,21 @@ public:
         return out;
     }
 
+    // Outputs of the product of two operands' digit planes that need the pipe.
+    int slice_guard(int Ap, int Bp, int64_t M, int64_t N, int64_t K) {
+        const int level = std::max({level_of(Ap), level_of(Bp), gfloor_}) + 1;
+        const int out = tensor(slice_guard_tiles(M, N) * 8 / pg_.esize, level);
+        Op op;
+        op.kind = OP_SLICE_GUARD;
+        op.level = level;
+        op.A = Ap; op.B = Bp; op.out = out;
+        op.gm = M; op.gn = N; op.gk = K;
+        op.bytes = (double)slice_mag_bytes(M + N, K);
+        use(Ap, level); use(Bp, level);
+        add(op);
+        return out;
+    }
+
     // C[m][n] = sum_k A(m,k) B(k,n); dot partner Cd -> scalar.
     int gemm(int A, int B, int64_t M, int64_t N, int64_t K, int64_t sam, int64_t sak,
              int64_t sbk, int64_t sbn, int Cd = -1) {
@@ -329,7 +345,9 @@ public:
             const int kb = slices ? slice_kmax(B, N, K, sbn, sbk) : -1;
             const int Ap = tc_split(A, M, K, sam, sak, ka, kb, slices);
             const int Bp = tc_split(B, N, K, sbn, sbk, kb, ka);
+            const int guard = slices ? slice_guard(Ap, Bp, M, N, K) : -1;
             int lv = std::max({level_of(Ap), level_of(Bp), gfloor_}) + 1;
+            if (slices) lv = std::max(lv, level_of(guard) + 1);
             if (Cd >= 0) lv = std::max(lv, level_of(Cd) + 1);
             const int o = Cd >= 0 ? scalar(lv) : tensor(M * N, lv);
             Op op;
@@ -338,6 +356,8 @@ public:
             op.A = Ap; op.B = Bp; op.C = Cd; op.out = o;
             op.A_src = A; op.B_src = B;
             op.gm = M; op.gn = N; op.gk = K;
+            op.sam = sam; op.sak = sak; op.sbk = sbk; op.sbn = sbn;
+            op.adj = guard;
             const int64_t kpad = slices ? kSliceKPad : 64;
             const int64_t ra = slices ? slice_row_pad(dt, true) : kTcRowPad, rb = slices ? slice_row_pad(dt, false) : kTcRowPad;
             op.Kp = (K + kpad - 1) / kpad * kpad;
@@ -347,6 +367,7 @@ public:
                        (double)M * N * pg_.esize;
             op.macs = (double)M * N * K;
             use(Ap, lv); use(Bp, lv); use(A, lv); use(B, lv);
+            if (slices) use(guard, lv);
             if (Cd >= 0) use(Cd, lv);
             add(op);
             return o;

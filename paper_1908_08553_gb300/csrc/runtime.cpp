@@ -34,7 +34,7 @@ int family_of(int kind) {
         case OP_ABSORB: return FAM_ABSORB;
         case OP_ABSORB_DOT: return FAM_ABSORB_DOT;
         case OP_ABSORB2: case OP_ABSORB2_DOT: return FAM_PAIR;
-        case OP_TC_SPLIT: case OP_SLICE_KMAX: case OP_SLICE_E: return FAM_OTHER;
+        case OP_TC_SPLIT: case OP_SLICE_KMAX: case OP_SLICE_E: case OP_SLICE_GUARD: return FAM_OTHER;
         case OP_GEMM: case OP_GEMM_DOT: return FAM_GEMM;
         case OP_TC_GEMM: case OP_TC_GEMM_DOT: return FAM_TC;
         default: return FAM_OTHER;
@@ -134,6 +134,12 @@ void materialize(tn_batch* b, char* base, std::vector<char>* tasks_out, std::vec
     auto slot_of = [&](int mi, int tid) -> int {
         return (int)(b->m[mi].slot_base + b->m[mi].pg->tensors[tid].slot);
     };
+    // after a product from digits: the pipe's kernel for the outputs its guard names.
+    // FP64 in 16 x 16 tiles: a few flagged ones spread over the SMs (128 x 128 of them on
+    // one SM would take 2 x 128 x 128 / 4 = 8192 cycles a term)
+    auto pipe_variant = [&](const Op& op) {
+        return b->dt == 0 ? kGemmSmall : gemm_variant(b->dt, op.gm, op.gn, op.gk, op.sam, op.sak, op.sbk, op.sbn);
+    };
     // partial region placement needs npart first: count dot tiles
     for (auto& kv : groups) {
         const int kind = std::get<1>(kv.first);
@@ -153,6 +159,11 @@ void materialize(tn_batch* b, char* base, std::vector<char>* tasks_out, std::vec
             else if (kind == OP_TC_GEMM_DOT) {
                 const int bn = std::get<4>(kv.first) % 1000;
                 npart += ((op.gm + 127) / 128) * ((op.gn + bn - 1) / bn);   // one partial per tile
+                if (op.slices) {                                           // and of the outputs left to the pipe
+                    int tn_;
+                    const int var = pipe_variant(op);
+                    npart += gemm_tiles_v(var, op.gm, op.gn, &tn_) * gemm_ksplit(var, true, op.gk);
+                }
             }
         }
     }
@@ -176,6 +187,34 @@ void materialize(tn_batch* b, char* base, std::vector<char>* tasks_out, std::vec
         tasks.resize(off + n);
         std::memcpy(tasks.data() + off, src, n);
         return off;
+    };
+    // C = A B (or its dot) on the pipe from tensors A and B
+    auto gemm_task = [&](const OpRef& r, int A, int B, bool dot, int variant, long long tile0) {
+        const Op& op = b->m[r.member].pg->ops[r.op];
+        GemmTask t{};
+        t.A = tensor_ptr(r.member, A);
+        t.B = tensor_ptr(r.member, B);
+        t.M = op.gm; t.N = op.gn; t.K = op.gk;
+        t.sam = op.sam; t.sak = op.sak; t.sbk = op.sbk; t.sbn = op.sbn;
+        t.slot_A = slot_of(r.member, A);
+        t.slot_B = slot_of(r.member, B);
+        t.slot_C = slot_of(r.member, op.out);
+        int tn_ = 0;
+        const long long ksp = gemm_ksplit(variant, dot, op.gk);
+        const long long nt = gemm_tiles_v(variant, op.gm, op.gn, &tn_) * ksp;
+        t.tiles_n = tn_;
+        t.ntiles = (int)nt;
+        t.ksplit = (int)ksp;
+        t.kslice = ksp > 1 ? kGemmKSlice : op.gk;
+        t.tile0 = tile0;
+        if (dot) {
+            t.Dm = tensor_ptr(r.member, op.C);
+            t.slot_D = slot_of(r.member, op.C);
+            t.partial = take_partial(nt);
+        } else {
+            t.C = tensor_ptr(r.member, op.out);
+        }
+        return t;
     };
     for (auto& kv : groups) {
         const int kind = std::get<1>(kv.first);
@@ -281,31 +320,29 @@ void materialize(tn_batch* b, char* base, std::vector<char>* tasks_out, std::vec
                 off = append(&t, sizeof(t));
                 tile += nt;
             } else if (kind == OP_GEMM || kind == OP_GEMM_DOT) {
-                GemmTask t{};
-                t.A = tensor_ptr(r.member, op.A);
-                t.B = tensor_ptr(r.member, op.B);
-                t.M = op.gm; t.N = op.gn; t.K = op.gk;
-                t.sam = op.sam; t.sak = op.sak; t.sbk = op.sbk; t.sbn = op.sbn;
-                t.slot_A = slot_of(r.member, op.A);
-                t.slot_B = slot_of(r.member, op.B);
-                t.slot_C = slot_of(r.member, op.out);
-                int tn_ = 0;
-                const long long ksp = gemm_ksplit(L.variant, kind == OP_GEMM_DOT, op.gk);
-                const long long nt = gemm_tiles_v(L.variant, op.gm, op.gn, &tn_) * ksp;
-                t.tiles_n = tn_;
-                t.ntiles = (int)nt;
-                t.ksplit = (int)ksp;
-                t.kslice = ksp > 1 ? kGemmKSlice : op.gk;
-                t.tile0 = tile;
-                if (kind == OP_GEMM_DOT) {
-                    t.Dm = tensor_ptr(r.member, op.C);
-                    t.slot_D = slot_of(r.member, op.C);
-                    t.partial = take_partial(nt);
-                } else {
-                    t.C = tensor_ptr(r.member, op.out);
-                }
+                const GemmTask t = gemm_task(r, op.A, op.B, kind == OP_GEMM_DOT, L.variant, tile);
                 off = append(&t, sizeof(t));
-                tile += nt;
+                tile += t.ntiles;
+            } else if (kind == OP_SLICE_GUARD) {
+                SliceGuardTask t{};
+                auto mags = [&](int id, long long rows, bool first) -> const void* {
+                    const char* p = static_cast<const char*>(tensor_ptr(r.member, id));
+                    const long long pad = slice_row_pad(b->dt, first), Rp = (rows + pad - 1) / pad * pad;
+                    const long long Kp = (op.gk + kSliceKPad - 1) / kSliceKPad * kSliceKPad;
+                    return p ? p + slice_planes(b->dt) * Rp * Kp * 2 + Rp * 4 : nullptr;
+                };
+                t.A = mags(op.A, op.gm, true);
+                t.B = mags(op.B, op.gn, false);
+                t.flags = static_cast<unsigned long long*>(tensor_ptr(r.member, op.out));
+                t.M = op.gm; t.N = op.gn; t.K = op.gk;
+                t.tiles_m = (op.gm + 127) / 128;
+                t.tiles_n = (int)((op.gn + 127) / 128);
+                t.ntiles = (int)slice_guard_tiles(op.gm, op.gn);
+                t.slot = slot_of(r.member, op.out);
+                t.least = slice_guard_least(b->dt, op.gk);
+                t.tile0 = tile;
+                off = append(&t, sizeof(t));
+                tile += t.ntiles;
             } else if (kind == OP_TC_SPLIT || kind == OP_SLICE_KMAX) {
                 TcSplitTask t{};
                 t.src = tensor_ptr(r.member, op.A);
@@ -353,6 +390,10 @@ void materialize(tn_batch* b, char* base, std::vector<char>* tasks_out, std::vec
                 const long long nt = t.tiles_m * t.tiles_n * ksp;
                 t.ntiles = (int)nt;
                 t.tile0 = tile;
+                if (op.slices) {
+                    t.flags = static_cast<const unsigned long long*>(tensor_ptr(r.member, op.adj));
+                    t.flags_n = (int)((op.gn + 127) / 128);
+                }
                 if (kind == OP_TC_GEMM_DOT) {
                     t.Dm = tensor_ptr(r.member, op.C);
                     t.slot_D = slot_of(r.member, op.C);
@@ -396,6 +437,32 @@ void materialize(tn_batch* b, char* base, std::vector<char>* tasks_out, std::vec
             }
         }
         b->launches.push_back(L);
+        if (L.variant < kSliceVariant || (kind != OP_TC_GEMM && kind != OP_TC_GEMM_DOT)) continue;
+        // products from digits: the outputs left to the pipe, one launch per kernel of its
+        std::map<int, std::vector<OpRef>> rest;
+        for (const OpRef& r : refs) rest[pipe_variant(b->m[r.member].pg->ops[r.op])].push_back(r);
+        for (const auto& vr : rest) {
+            Launch P;
+            P.kind = kind == OP_TC_GEMM_DOT ? OP_GEMM_DOT : OP_GEMM;
+            P.level = L.level;
+            P.dt = b->dt;
+            P.variant = vr.first;
+            P.ntasks = (int)vr.second.size();
+            align_group();
+            P.task_off = tasks.size();
+            long long tile0 = 0;
+            for (const OpRef& r : vr.second) {
+                const Op& op = b->m[r.member].pg->ops[r.op];
+                GemmTask t = gemm_task(r, op.A_src, op.B_src, kind == OP_TC_GEMM_DOT, vr.first, tile0);
+                t.flags = static_cast<const unsigned long long*>(tensor_ptr(r.member, op.adj));
+                t.flags_n = (int)((op.gn + 127) / 128);
+                t.slot_flags = slot_of(r.member, op.adj);
+                append(&t, sizeof(t));
+                tile0 += t.ntiles;
+            }
+            P.nblocks = tile0;
+            b->launches.push_back(P);
+        }
     }
     // const-one tensors
     for (int mi = 0; mi < (int)b->m.size(); ++mi) {
@@ -663,6 +730,9 @@ cudaError_t issue(tn_batch* b, cudaStream_t st, std::vector<std::pair<cudaEvent_
                 break;
             case OP_SLICE_E:
                 e = launch_slice_e(static_cast<const AbsorbTask*>(tp), L.ntasks, st);
+                break;
+            case OP_SLICE_GUARD:
+                e = launch_slice_guard(static_cast<const SliceGuardTask*>(tp), L.ntasks, L.nblocks, slots, status, st);
                 break;
             case OP_SLICE_KMAX:
                 e = launch_slice_kmax(L.dt, static_cast<const TcSplitTask*>(tp), L.ntasks, L.nblocks, st);

@@ -79,6 +79,7 @@ enum OpKind {
     OP_TC_SPLIT,      // FP32 / FP64 operand -> tiled BF16 planes (tensor-core input)
     OP_SLICE_KMAX,    // FP64 / FP32 operand -> largest exponent of each of its terms (balances OP_TC_SPLIT)
     OP_SLICE_E,       // FP64 layer factors -> digit planes of the D = 3 double-layer site matrix
+    OP_SLICE_GUARD,   // digit planes of a product's operands -> its outputs that need the pipe
     OP_TC_GEMM,       // C = A B^T on tensor cores from split planes
     OP_TC_GEMM_DOT,   // scalar = <A B^T, C> on tensor cores
     OP_ABSORB2,       // out = absorb(absorb(in, E), E2): two steps of one frame row

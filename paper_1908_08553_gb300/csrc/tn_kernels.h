@@ -62,6 +62,10 @@ struct GemmTask {
     int tiles_n, ntiles;
     int ksplit;           // tiles along k (dot mode: one FP64 partial each)
     int slot_A, slot_B, slot_C, slot_D;
+    // after a product from digits (else null): only the tiles its guard names
+    // (SliceGuardTask::flags), their dot added to the slot's
+    const unsigned long long* flags;
+    int flags_n, slot_flags;
 };
 
 // k-slice of the products fused with a dot: partial sums of at most this
@@ -150,6 +154,22 @@ struct TcGemmTask {
     int tiles_n, ntiles;
     int ksplit;
     int slot_A, slot_B, slot_C, slot_D;   // slots of the FP32 sources / result
+    const unsigned long long* flags;      // digit planes: outputs left to the pipe (SliceGuardTask)
+    int flags_n, pad;
+};
+
+// Guard of a product from digit planes (slice_gemm.cu): which outputs of C have
+// terms too small for the digits.  One word per 128 x 128 tile (flags_n of them
+// per row of tiles): bit 8 i + j for rows 16 i.. and columns 16 j.. of the tile.
+struct SliceGuardTask {
+    const void* A;                // magnitude planes (slice_mag_bytes) of both operands
+    const void* B;
+    unsigned long long* flags;
+    long long M, N, K;
+    long long tile0, tiles_m;
+    int tiles_n, ntiles;
+    int slot;                     // slot of the flags: maxbits is raised if any bit is set
+    float least;                  // outputs whose terms' magnitudes sum to less are flagged
 };
 
 // One bond of an imaginary-time two-body update (Sec. 5, Fig. 3): sites i and j
@@ -254,12 +274,19 @@ constexpr int kTcChunk = 32;
 // (slice_gemm.cu).  An operand is kept as kSlicePlanes (FP64) or kSlicePlanes32
 // (FP32) BF16 planes of Rp x Kp (Rp rounded up to slice_row_pad, Kp to
 // kSliceKPad), then one int32 exponent per row (TcSplitTask::plane_bytes,
-// TcGemmTask::a_/b_plane_bytes: the planes' bytes).
+// TcGemmTask::a_/b_plane_bytes: the planes' bytes), then the magnitudes as one
+// E5M2 plane for the guard (Kp rounded up to 32).
 constexpr int kSlicePlanes = 7, kSlicePlanes32 = 3;
 constexpr long long kSliceKPad = 16;
 inline int slice_planes(int dt) { return dt == 0 ? kSlicePlanes : kSlicePlanes32; }
 inline long long slice_row_pad(int dt, bool first) { return dt == 0 || first ? 128 : 256; }
+inline long long slice_mag_bytes(long long Rp, long long K) { return Rp * ((K + 31) / 32 * 32); }
 bool slice_ok(bool f64, long long M, long long N, long long K);
+// The guard: launched between the splits and the product.
+inline long long slice_guard_tiles(long long M, long long N) { return ((M + 127) / 128) * ((N + 127) / 128); }
+float slice_guard_least(int dt, long long K);
+cudaError_t launch_slice_guard(const SliceGuardTask* tasks, int ntasks, long long nblocks, Slot* slots, int* status,
+                               cudaStream_t st);
 long long slice_split_tiles(long long Rp);
 cudaError_t launch_slice_split(int dt, const TcSplitTask* tasks, int ntasks, long long nblocks, cudaStream_t st);
 // The largest exponent of each of the Kp terms of an operand (TcSplitTask::dst: Kp int32).

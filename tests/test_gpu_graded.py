@@ -1,0 +1,125 @@
+"""States whose boundary tensors span many binades inside one row or column: the
+digit products (program choice bit 3) have to be as good as the multiply-add
+pipes (bit 3 cleared) there too."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1908_08553_gb300 import inputs, tn
+
+pytestmark = pytest.mark.gpu
+E = tn.TN_WORK_ENERGY
+NO_PLANES = 15 & ~8
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    import torch
+    torch.cuda.init()
+    c = tn.tn_ctx_create(0, 0)
+    yield c
+    tn.tn_ctx_destroy(c)
+
+
+def _full(ctx, L, W, D, A, knobs, prec):
+    """log2 of the norm as (mantissa, exponent), then <X>, <ZZ>, <Z>."""
+    tn.tn_autotune_set(L, W, D, prec, E, knobs)
+    lat = tn.tn_create_lattice(ctx, L, W, D)
+    try:
+        tn.tn_set_site_tensors(lat, A)
+        r, sx, zz, sz, _ = tn.tn_energy_full(lat, 1.0, 3.04, prec, tn.TN_SCHED_AUTO, L, W)
+        return (r.norm.mant, r.norm.exp2), sx, zz, sz
+    finally:
+        tn.tn_destroy_lattice(lat)
+        tn.tn_autotune_clear()
+
+
+def _off(norm, ref):
+    return abs(norm[0] / ref[0] * 2.0 ** (norm[1] - ref[1]) - 1.0)
+
+
+def seam_ising(L, W, beta):
+    """Classical Ising model as a PEPS (the norm is its partition function): legs carry
+    spins, all couplings +1 but -1 on the lower half's middle column of bonds, so the
+    two halves prefer different configurations on the cut between them.  All entries
+    are non-negative: sums of products lose nothing to cancellation."""
+    w = np.exp(0.5 * beta * np.array([[1.0, -1.0], [-1.0, 1.0]]))
+    one = np.ones((1, 2))
+    sites = []
+    for r in range(L):
+        for c in range(W):
+            u, l, dn, rt = inputs.site_dims(L, W, 2, r, c)
+            up = w if u > 1 else one
+            anti = r >= L // 2 and c == W // 2
+            left = (1.0 / w if anti else w) if l > 1 else one
+            A = np.zeros((2, u, l, dn, rt))
+            for p in range(2):
+                A[p, :, :, p if dn > 1 else 0, p if rt > 1 else 0] = np.outer(up[:, p], left[:, p])
+            sites.append(A.ravel())
+    return np.concatenate(sites)
+
+
+# The products' operands are non-negative, so every sum keeps its relative accuracy: in
+# FP64 three ring products and 64 absorptions of at most 256 + 16 roundings each stay
+# below (3 * 256 + 64 * 16) 2^-53 = 2e-13 if all of them pull one way.
+@pytest.mark.parametrize("beta", [1.5, 2.0])
+def test_frustrated_seam_fp64(ctx, beta):
+    L = W = 8
+    A = seam_ising(L, W, beta)
+    ref = oracle.norm(L, W, 2, A)
+    obs = oracle.observables(L, W, 2, A, with_z=True)
+    for knobs in (NO_PLANES, 15):
+        norm, sx, zz, sz = _full(ctx, L, W, 2, A, knobs, tn.TN_FP64)
+        assert _off(norm, ref) <= 1e-12, knobs
+        for x, y in ((sx, obs.sx), (zz, obs.szsz), (sz, obs.sz)):
+            assert np.max(np.abs(x - y)) <= 1e-12, knobs
+
+
+# FP32: a product's roundings add up to sqrt(1024) 2^-24 = 2e-6 of a sum of non-negative
+# terms, a digit product's to at most 2e-6; three of them and 100 absorptions of 4e-7
+# (0.24e-6 sqrt(100)) give 1.2e-5 at most.
+@pytest.mark.parametrize("beta", [0.75, 1.0])
+def test_frustrated_seam_fp32(ctx, beta):
+    L = W = 10
+    A = seam_ising(L, W, beta)
+    ref, _, zz64, _ = _full(ctx, L, W, 2, A, NO_PLANES, tn.TN_FP64)
+    for knobs in (NO_PLANES, 15):
+        norm, _, zz, _ = _full(ctx, L, W, 2, A, knobs, tn.TN_FP32)
+        assert _off(norm, ref) <= 1.2e-5, knobs
+        assert np.max(np.abs(zz - zz64)) <= 1.2e-5, knobs
+
+
+def parity_state(L, W, eps, seed):
+    """Random D = 2 state that conserves the parity of its legs up to entries of size eps:
+    nearly block-diagonal boundary tensors, and <X> (odd) of the order of eps."""
+    sites = []
+    for t in inputs.split_sites(inputs.random_lattice(L, W, 2, seed), L, W, 2):
+        odd = np.indices(t.shape).sum(0) % 2 == 1
+        sites.append(np.where(odd, eps * t, t).ravel())
+    return np.concatenate(sites)
+
+
+# <X> is a sum of terms eps times those of the norm, so it keeps a relative accuracy
+# of its own; the pipe's error is the yardstick (a handful of roundings either way),
+# with 2^-20 of the largest <X> for the products' own.
+@pytest.mark.parametrize("L,W,prec,ulp,eps", [(8, 8, tn.TN_FP64, 2.0 ** -46, 2.0 ** -10),
+                                              (10, 10, tn.TN_FP32, 2.0 ** -17, 2.0 ** -10),
+                                              (10, 10, tn.TN_FP32, 2.0 ** -17, 2.0 ** -20)])
+def test_nearly_block_diagonal(ctx, L, W, prec, ulp, eps):
+    A = parity_state(L, W, eps, 4100)
+    ref = (oracle.observables(L, W, 2, A).sx if prec == tn.TN_FP64
+           else _full(ctx, L, W, 2, A, NO_PLANES, tn.TN_FP64)[1])
+    pipe, dig = (_full(ctx, L, W, 2, A, k, prec)[1] for k in (NO_PLANES, 15))
+    bound = 4 * np.max(np.abs(pipe - ref)) + ulp * np.max(np.abs(ref))
+    assert np.max(np.abs(dig - ref)) <= bound
+
+
+# exactly conserved parity: half of every boundary tensor is structurally zero
+def test_conserved_parity(ctx):
+    L, W = 8, 8
+    A = parity_state(L, W, 0.0, 4200)
+    obs = oracle.observables(L, W, 2, A, with_z=True)
+    _, sx, zz, sz = _full(ctx, L, W, 2, A, 15, tn.TN_FP64)
+    assert np.all(sx == 0.0)
+    for x, y in ((zz, obs.szsz), (sz, obs.sz)):
+        assert np.max(np.abs(x - y)) <= 1e-12
