@@ -89,11 +89,11 @@ def test_frustrated_seam_fp32(ctx, beta):
         assert np.max(np.abs(zz - zz64)) <= 1.2e-5, knobs
 
 
-def parity_state(L, W, eps, seed):
-    """Random D = 2 state that conserves the parity of its legs up to entries of size eps:
+def parity_state(L, W, eps, seed, D=2):
+    """Random state that conserves the parity of its legs up to entries of size eps:
     nearly block-diagonal boundary tensors, and <X> (odd) of the order of eps."""
     sites = []
-    for t in inputs.split_sites(inputs.random_lattice(L, W, 2, seed), L, W, 2):
+    for t in inputs.split_sites(inputs.random_lattice(L, W, D, seed), L, W, D):
         odd = np.indices(t.shape).sum(0) % 2 == 1
         sites.append(np.where(odd, eps * t, t).ravel())
     return np.concatenate(sites)
@@ -102,9 +102,8 @@ def parity_state(L, W, eps, seed):
 # <X> is a sum of terms eps times those of the norm, so it keeps a relative accuracy
 # of its own; the pipe's error is the yardstick (a handful of roundings either way),
 # with 2^-20 of the largest <X> for the products' own.
-@pytest.mark.parametrize("L,W,prec,ulp,eps", [(8, 8, tn.TN_FP64, 2.0 ** -46, 2.0 ** -10),
-                                              (10, 10, tn.TN_FP32, 2.0 ** -17, 2.0 ** -10),
-                                              (10, 10, tn.TN_FP32, 2.0 ** -17, 2.0 ** -20)])
+@pytest.mark.parametrize("L,W,prec,ulp", [(8, 8, tn.TN_FP64, 2.0 ** -46), (10, 10, tn.TN_FP32, 2.0 ** -17)])
+@pytest.mark.parametrize("eps", [2.0 ** -10, 2.0 ** -20])
 def test_nearly_block_diagonal(ctx, L, W, prec, ulp, eps):
     A = parity_state(L, W, eps, 4100)
     ref = (oracle.observables(L, W, 2, A).sx if prec == tn.TN_FP64
@@ -123,3 +122,40 @@ def test_conserved_parity(ctx):
     assert np.all(sx == 0.0)
     for x, y in ((zz, obs.szsz), (sz, obs.sz)):
         assert np.max(np.abs(x - y)) <= 1e-12
+
+
+# D = 3: absorptions of 81 and 9 legs from digits; <X> against the oracle's as above
+@pytest.mark.parametrize("eps", [2.0 ** -10, 2.0 ** -18, 2.0 ** -26])
+def test_nearly_block_diagonal_d3(ctx, eps):
+    L, W = 4, 5
+    A = parity_state(L, W, eps, 4300, 3)
+    ref = oracle.observables(L, W, 3, A).sx
+    pipe, dig = (_full(ctx, L, W, 3, A, k, tn.TN_FP64)[1] for k in (NO_PLANES, 15))
+    assert np.max(np.abs(dig - ref)) <= 4 * np.max(np.abs(pipe - ref)) + 2.0 ** -46 * np.max(np.abs(ref))
+
+
+# one end of every bond padded: leg index D - 1 has zeros on the right / lower site and
+# entries 2^g above the others on the left / upper one.  The state is the one of bond
+# dimension D - 1; the inputs' largest entries meet empty rows of the site matrices.
+# 4 x 5 sites of at most 81 roundings a step: sqrt(20 * 81) 2^-53 = 4.5e-15 on a sum,
+# 10 times that on the ratios.
+@pytest.mark.parametrize("D", [2, 3])
+@pytest.mark.parametrize("g", [6, 9, 30])
+def test_bonds_padded_at_one_end(ctx, D, g):
+    L, W = 4, 5
+    sites = [np.array(t) for t in inputs.split_sites(inputs.random_lattice(L, W, D, 4400 + D), L, W, D)]
+    for t in sites:
+        for axis in (1, 2):
+            if t.shape[axis] > 1:
+                np.moveaxis(t, axis, 0)[D - 1] = 0.0
+        for axis in (3, 4):
+            if t.shape[axis] > 1:
+                np.moveaxis(t, axis, 0)[D - 1] *= 2.0 ** g
+    A = inputs.join_sites(sites)
+    small = inputs.join_sites([t[:, :max(1, t.shape[1] - (t.shape[1] > 1)), :max(1, t.shape[2] - (t.shape[2] > 1)),
+                                 :max(1, t.shape[3] - (t.shape[3] > 1)), :max(1, t.shape[4] - (t.shape[4] > 1))]
+                               for t in sites])
+    obs = oracle.observables(L, W, D - 1, small, with_z=True)
+    _, sx, zz, sz = _full(ctx, L, W, D, A, 15, tn.TN_FP64)
+    for x, y in ((sx, obs.sx), (zz, obs.szsz), (sz, obs.sz)):
+        assert np.max(np.abs(x - y)) <= 5e-14
