@@ -159,3 +159,28 @@ def test_bonds_padded_at_one_end(ctx, D, g):
     _, sx, zz, sz = _full(ctx, L, W, D, A, 15, tn.TN_FP64)
     for x, y in ((sx, obs.sx), (zz, obs.szsz), (sz, obs.sz)):
         assert np.max(np.abs(x - y)) <= 5e-14
+
+
+# an output of a product may lie as far below its operands' largest entries as FP32
+# reaches: in the upper half, column 2's sites carry one sector along the cut, 0 with
+# weight 1 or 1 with a small one, column 3's sector 2 with weight 1 or 1 with a small
+# one; only sector 1 crosses, so that half's ring product is 2^-112 of its operands'
+# largest entries, in rows and columns of its own.  FP32 keeps 2^-24 of each of the
+# norm's 729 x 729 products of random sign: 2e-5 of a norm 1/300 of its terms' size at
+# worst.
+def test_fp32_products_of_small_rows_and_columns(ctx):
+    L = W = 6
+    D, f = 3, 2.0 ** -9.3
+    sites = [np.array(t) for t in inputs.split_sites(inputs.random_lattice(L, W, D, 4500), L, W, D)]
+    for r in range(L // 2):
+        for c, legs, weight in ((2, (1, 3, 4), (1.0, f, 0.0)), (3, (1, 3, 2), (0.0, f, 1.0))):
+            t = sites[r * W + c]
+            idx = np.indices(t.shape)
+            cut = idx[legs[2]]
+            same = [idx[leg] == cut for leg in legs[:2] if t.shape[leg] > 1]
+            sites[r * W + c] = t * np.array(weight)[cut] * np.logical_and.reduce(same)
+    A = inputs.join_sites(sites)
+    ref = oracle.norm(L, W, D, A)
+    for knobs in (NO_PLANES, 15):
+        norm, _, _, _ = _full(ctx, L, W, D, A, knobs, tn.TN_FP32)
+        assert _off(norm, ref) <= 2e-5, knobs
