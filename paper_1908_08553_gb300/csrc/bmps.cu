@@ -347,8 +347,10 @@ cudaError_t launch_bmps(int dt, const BmpsTask* tasks, int ntasks, int D, int ch
     const long long most = 104 * 1024, one = 200 * 1024;
     const int bytes = (int)(need <= most ? need : need <= one ? need : most);
     const int elems = bytes / (int)es;
-    const cudaError_t e = dt == 0 ? cudaFuncSetAttribute(k_bmps<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes)
-                                  : cudaFuncSetAttribute(k_bmps<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    // the limit belongs to the function, not to the call: always the largest, so that calls of
+    // other threads cannot lower it between here and the launch
+    const cudaError_t e = dt == 0 ? cudaFuncSetAttribute(k_bmps<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)one)
+                                  : cudaFuncSetAttribute(k_bmps<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)one);
     if (e != cudaSuccess) return e;
     if (dt == 0) k_bmps<double><<<ntasks, kBmpsThreads, bytes, st>>>(tasks, elems);
     else k_bmps<float><<<ntasks, kBmpsThreads, bytes, st>>>(tasks, elems);

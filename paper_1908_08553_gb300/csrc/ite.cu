@@ -209,8 +209,10 @@ cudaError_t launch_ite_bonds(double* A, const IteBondTask* tasks, int ntasks, in
                              cudaStream_t st) {
     if (ntasks <= 0) return cudaSuccess;
     // ws_max: the largest bond's workspace (doubles); at D <= 3 it fits shared memory
-    const int bytes = ws_max * 8 <= 100 * 1024 ? ws_max * 8 : 0;
-    const cudaError_t e = cudaFuncSetAttribute(k_ite_bond, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    constexpr int most = 100 * 1024;
+    const int bytes = ws_max * 8 <= most ? ws_max * 8 : 0;
+    // the limit belongs to the function, not to the call (other threads' lattices): always the largest
+    const cudaError_t e = cudaFuncSetAttribute(k_ite_bond, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     if (e != cudaSuccess) return e;
     k_ite_bond<<<ntasks, kIteThreads, bytes, st>>>(A, tasks, ntasks, ws, g[0], g[1], g[2], g[3], chi_max, eps, kept,
                                                    max_disc, bytes / 8);
