@@ -341,11 +341,14 @@ const void* bmps_module_anchor() { return reinterpret_cast<const void*>(&k_bmps<
 cudaError_t launch_bmps(int dt, const BmpsTask* tasks, int ntasks, int D, int chi, cudaStream_t st) {
     if (ntasks <= 0) return cudaSuccess;
     // shared memory for the largest SVD of this shape, B columns of d B rows and
-    // V, as far as two blocks on an SM allow (larger ones stay in the workspace)
+    // V, when it fits (larger ones stay in the workspace, all of them: with room for only
+    // the small ones a block displaces the L1 cache the others live on, 5x5 D=3 chi=9 in
+    // FP32 147.6 ms against 86.7).  FP32 also at one block an SM (8x8 chi=24 172 against
+    // 181 ms); FP64 gains nothing by that (chi=16 1363 against 1356).
     const long long B = bmps_bond_max(D, chi), d = (long long)D * D, es = dt == 0 ? 8 : 4;
     const long long need = B * ((d * B | 1) + (B | 1)) * es;
     const long long most = 104 * 1024, one = 200 * 1024;
-    const int bytes = (int)(need <= most ? need : need <= one ? need : most);
+    const int bytes = (int)(need <= (dt == 0 ? most : one) ? need : 0);
     const int elems = bytes / (int)es;
     // the limit belongs to the function, not to the call: always the largest, so that calls of
     // other threads cannot lower it between here and the launch
