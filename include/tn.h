@@ -415,7 +415,9 @@ tn_status tn_ite_init_product(tn_lattice *lat);
  * tensors hold the evolved state on return.  Device memory for the program
  * buffers and an SVD workspace (m n + n^2 doubles per bond of a class, m, n
  * <= 2 D^3) comes from the context's budget.  TN_ERR_INVALID for bad
- * parameters, TN_ERR_NUMERIC for a non-finite energy. */
+ * parameters, TN_ERR_NUMERIC for a non-finite energy, TN_ERR_TIMEOUT (and the
+ * lattice's tensors as they were) if a bounded device wait gave up in any of
+ * its norms or energies. */
 tn_status tn_ite_run(tn_lattice *lat, const tn_ite_params *params, double *energies, int *bond_dims,
                      double *max_discarded);
 
@@ -521,7 +523,8 @@ tn_status tn_wait_selfcheck(tn_ctx *ctx, double limit_ms, int *expired);
 tn_status tn_peak_probe(tn_ctx *ctx, int dtype, double *tflops);
 /* Host-side fault injection (no counterpart in the paper; failure detection):
  * the next `count` batch runs of this context -- served batches, tn_energy and
- * the other blocking calls, tn_batch_run -- have their status word set after
+ * the other blocking calls (tn_ite_run's norms and energies and tn_autotune's
+ * runs among them), tn_batch_run -- have their status word set after
  * their kernels are queued, exactly as a bounded device wait that ran out
  * would set it, so the error path (TN_ERR_TIMEOUT from tn_poll / tn_wait, the
  * blocking calls and tn_batch_results_host) can be tested without disturbing

@@ -40,8 +40,10 @@ __global__ void k_ite_one_body(double* __restrict__ A, const long long* __restri
 
 // Multiply the state by 2^(-log2 N / (2 n_sites)) per site, N the norm read from
 // the norm program's result row (entry 1: log2 <Psi|Psi>), so <Psi|Psi> -> 1.
+// That run's status word is kept in `failed`: the next run clears it.
 __global__ void k_ite_scale(double* __restrict__ A, long long n, const double* __restrict__ log2norm,
-                            int nsites) {
+                            int nsites, const int* __restrict__ status, int* __restrict__ failed) {
+    if (blockIdx.x == 0 && threadIdx.x == 0 && *status) *failed = 1;
     const double f = exp2(-log2norm[0] / (2.0 * nsites));
     for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x)
         A[k] *= f;
@@ -197,10 +199,11 @@ cudaError_t launch_ite_one_body(double* A, const long long* site_off, int nsites
     return cudaGetLastError();
 }
 
-cudaError_t launch_ite_scale(double* A, long long n, const double* log2norm, int nsites, cudaStream_t st) {
+cudaError_t launch_ite_scale(double* A, long long n, const double* log2norm, int nsites, const int* status,
+                             int* failed, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     const long long blocks = (n + 255) / 256 < 1024 ? (n + 255) / 256 : 1024;
-    k_ite_scale<<<(unsigned)blocks, 256, 0, st>>>(A, n, log2norm, nsites);
+    k_ite_scale<<<(unsigned)blocks, 256, 0, st>>>(A, n, log2norm, nsites, status, failed);
     return cudaGetLastError();
 }
 

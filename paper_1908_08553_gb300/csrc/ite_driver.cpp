@@ -10,6 +10,7 @@
 // read once at the end.  Bonds are updated in four classes of disjoint bonds
 // (horizontal with even left column, odd, vertical with even upper row, odd),
 // one launch per class, one block per bond.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -178,7 +179,9 @@ tn_status tn_ite_run(tn_lattice* lat, const tn_ite_params* prm, double* energies
         const size_t b_kept = b_tasks + ntask_all * sizeof(IteBondTask);
         const size_t b_disc = (b_kept + (size_t)ntask_all * sizeof(int) + 15) / 16 * 16;
         const size_t b_en = b_disc + 16;
-        const size_t b_ws = (b_en + (size_t)std::max(n_e, 1) * sizeof(double) + 255) / 256 * 256;
+        // status words: entry 0 of the norms (sticky), then of each energy
+        const size_t b_st = b_en + (size_t)std::max(n_e, 1) * sizeof(double);
+        const size_t b_ws = (b_st + (size_t)(n_e + 1) * sizeof(int) + 255) / 256 * 256;
         const size_t total = b_ws + (size_t)ws_need * sizeof(double);
         DevBuf buf;
         st = buf.alloc(ctx, total);
@@ -195,6 +198,7 @@ tn_status tn_ite_run(tn_lattice* lat, const tn_ite_params* prm, double* energies
             e = cudaMemcpyAsync(base + b_tasks, htasks.data(), htasks.size() * sizeof(IteBondTask),
                                 cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess) e = cudaMemsetAsync(base + b_disc, 0, 16, s);
+        if (e == cudaSuccess) e = cudaMemsetAsync(base + b_st, 0, (size_t)(n_e + 1) * sizeof(int), s);
         if (e == cudaSuccess)
             e = cudaMemcpyAsync(dA, lat->host.data(), (size_t)nel * sizeof(double), cudaMemcpyHostToDevice, s);
         if (e != cudaSuccess) return cuda_status(e, "ITE upload");
@@ -204,6 +208,8 @@ tn_status tn_ite_run(tn_lattice* lat, const tn_ite_params* prm, double* energies
         auto* d_disc = reinterpret_cast<unsigned long long*>(base + b_disc);
         double* d_en = reinterpret_cast<double*>(base + b_en);
         double* d_ws = reinterpret_cast<double*>(base + b_ws);
+        int* d_st = reinterpret_cast<int*>(base + b_st);
+        const int* d_norm_st = reinterpret_cast<const int*>(bN->buf + bN->lay.status_off);
 
         const double a = prm->gamma * prm->dtau / 2.0;
         const double g1[4] = {std::cosh(a), std::sinh(a), std::sinh(a), std::cosh(a)};
@@ -212,7 +218,7 @@ tn_status tn_ite_run(tn_lattice* lat, const tn_ite_params* prm, double* energies
         auto normalise = [&]() -> tn_status {
             tn_status r = batch_run(bN, s);
             if (r != TN_OK) return r;
-            return cuda_status(launch_ite_scale(dA, nel, d_log2n, nsites, s), "ITE scale");
+            return cuda_status(launch_ite_scale(dA, nel, d_log2n, nsites, d_norm_st, d_st, s), "ITE scale");
         };
         int ek = 0;
         for (int step = 1; step <= prm->steps; ++step) {
@@ -234,6 +240,9 @@ tn_status tn_ite_run(tn_lattice* lat, const tn_ite_params* prm, double* energies
                 if (e != cudaSuccess) return cuda_status(e, "ITE energy input");
                 if ((st = batch_run(bE, s)) != TN_OK) return st;
                 e = cudaMemcpyAsync(d_en + ek, bE->buf + bE->lay.res_off, sizeof(double), cudaMemcpyDeviceToDevice, s);
+                if (e == cudaSuccess)
+                    e = cudaMemcpyAsync(d_st + 1 + ek, bE->buf + bE->lay.status_off, sizeof(int),
+                                        cudaMemcpyDeviceToDevice, s);
                 if (e != cudaSuccess) return cuda_status(e, "ITE energy copy");
                 ++ek;
             }
@@ -241,7 +250,10 @@ tn_status tn_ite_run(tn_lattice* lat, const tn_ite_params* prm, double* energies
         std::vector<int> hkept(std::max<size_t>(ntask_all, 1));
         unsigned long long hdisc = 0;
         std::vector<double> hen(std::max(n_e, 1));
-        e = cudaMemcpyAsync(lat->host.data(), dA, (size_t)nel * sizeof(double), cudaMemcpyDeviceToHost, s);
+        std::vector<double> hA((size_t)nel);
+        std::vector<int> hst((size_t)n_e + 1);
+        e = cudaMemcpyAsync(hA.data(), dA, (size_t)nel * sizeof(double), cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(hst.data(), d_st, hst.size() * sizeof(int), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess && ntask_all)
             e = cudaMemcpyAsync(hkept.data(), d_kept, ntask_all * sizeof(int), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaMemcpyAsync(&hdisc, d_disc, sizeof(hdisc), cudaMemcpyDeviceToHost, s);
@@ -249,6 +261,12 @@ tn_status tn_ite_run(tn_lattice* lat, const tn_ite_params* prm, double* energies
             e = cudaMemcpyAsync(hen.data(), d_en, (size_t)n_e * sizeof(double), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return cuda_status(e, "ITE read-back");
+        for (int v : hst)
+            if (v) {                    // the state is left as it was
+                set_error("a bounded wait in a kernel timed out");
+                return TN_ERR_TIMEOUT;
+            }
+        std::copy(hA.begin(), hA.end(), lat->host.begin());
         if (energies)
             for (int k = 0; k < ek; ++k) energies[k] = hen[k];
         if (bond_dims) {

@@ -318,7 +318,8 @@ cudaError_t launch_slice_gemm(int dt, bool dot, const TcGemmTask* tasks, int nta
 // 2 x 2 gate; bonds: the diagonal two-body gate g[p_i][p_j]).
 cudaError_t launch_ite_one_body(double* A, const long long* site_off, int nsites, const double g[4],
                                 cudaStream_t st);
-cudaError_t launch_ite_scale(double* A, long long n, const double* log2norm, int nsites, cudaStream_t st);
+cudaError_t launch_ite_scale(double* A, long long n, const double* log2norm, int nsites, const int* status,
+                             int* failed, cudaStream_t st);
 cudaError_t launch_ite_bonds(double* A, const IteBondTask* tasks, int ntasks, int ws_max, double* ws,
                              const double g[4], int chi_max, double eps, int* kept, unsigned long long* max_disc,
                              cudaStream_t st);
