@@ -49,6 +49,16 @@ std::vector<int> candidates(int D, tn_precision prec, tn_work work) {
     return out;
 }
 
+// Waits for the last run; a bounded wait that gave up in it is an error (its time means nothing).
+tn_status finished(tn_batch* b, const char* what) {
+    int status = 0;
+    cudaError_t e = cudaMemcpyAsync(&status, b->buf + b->lay.status_off, sizeof(int), cudaMemcpyDeviceToHost, b->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+    if (e != cudaSuccess) return cuda_status(e, what);
+    if (status) { set_error("a bounded wait in a kernel timed out"); return TN_ERR_TIMEOUT; }
+    return TN_OK;
+}
+
 }  // namespace
 
 Knobs tuned_knobs(int L, int W, int D, tn_precision prec, tn_work work) {
@@ -107,7 +117,7 @@ tn_status tn_autotune(tn_ctx* ctx, int n, const int* L, const int* W, const int*
                 st = tn_batch_fill_random(b, 12345);
                 for (int k = 0; k < copies && st == TN_OK; ++k) { b->h_final[k].J = 1.0; b->h_final[k].h = hs[k]; }
                 if (st == TN_OK) st = batch_run(b, b->stream);     // capture + warm-up
-                if (st == TN_OK) st = cuda_status(cudaStreamSynchronize(b->stream), "autotune warm-up");
+                if (st == TN_OK) st = finished(b, "autotune warm-up");
                 float ms = 0.0f;
                 if (st == TN_OK) {
                     cudaEventRecord(e0, b->stream);
@@ -115,6 +125,7 @@ tn_status tn_autotune(tn_ctx* ctx, int n, const int* L, const int* W, const int*
                     cudaEventRecord(e1, b->stream);
                     if (st == TN_OK) st = cuda_status(cudaEventSynchronize(e1), "autotune timing");
                     if (st == TN_OK) cudaEventElapsedTime(&ms, e0, e1);
+                    if (st == TN_OK) st = finished(b, "autotune timing");
                 }
                 batch_destroy(b);
                 if (st != TN_OK) { result = st; break; }

@@ -35,3 +35,18 @@ def test_evolution_reports_a_timed_out_wait(ctx, count, every):
         assert np.array_equal(got, tn.tn_ite_run(lat, L, W, 1.0, 3.04, 0.05, 1, D, 1e-12, 1)[0])
     finally:
         tn.tn_destroy_lattice(lat)
+
+
+def test_autotuner_reports_a_timed_out_wait(ctx):
+    tn.tn_autotune_clear()
+    try:
+        for count in (1, 2):        # the warm-up; the warm-up and the timed run
+            tn.tn_ctx_inject_wait_timeout(ctx, count)
+            with pytest.raises(tn.TNError) as e:
+                tn.tn_autotune(ctx, [4], [4], [2], tn.TN_FP64, reps=1)
+            assert e.value.status == tn.TN_ERR_TIMEOUT
+            tn.tn_ctx_inject_wait_timeout(ctx, 0)
+        assert not tn.tn_autotune_lookup(4, 4, 2, tn.TN_FP64)["tuned"]
+    finally:
+        tn.tn_ctx_inject_wait_timeout(ctx, 0)
+        tn.tn_autotune_clear()
