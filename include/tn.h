@@ -213,8 +213,11 @@ tn_status tn_site_expectations(tn_lattice *lat, tn_precision prec, int op, doubl
  * budget left, this call and every other observable call on the lattice
  * (tn_expectation, tn_site_expectations, tn_bond_correlators,
  * tn_pair_correlators) take the recompute form (program choice bit 5: the
- * same values, bit for bit, in less memory); TN_ERR_OVER_BUDGET if that does
- * not fit either.  Served jobs do not fall back (tn_submit). */
+ * same values, bit for bit, in less memory), in FP64 and FP32 then the products
+ * without digit planes (bit 3 cleared: the same values to rounding, not bit
+ * for bit), then both; TN_ERR_OVER_BUDGET if nothing fits.  tn_batch_create and
+ * tn_ite_run fall back to the products without digit planes only, tn_submit
+ * and the members of a group as described there. */
 tn_status tn_energy(tn_lattice *lat, double J, double h, tn_precision prec, tn_result *out);
 /* Nearest-neighbour two-site correlators <A_i B_j> (blocking, AUTO schedule):
  * one Pauli operator on each site of every bond, A = op_a on the bond's first
@@ -279,7 +282,10 @@ tn_status tn_batch_launch_count(const tn_batch *b, int64_t *n);
  * tables); the launches of all passes are captured into ONE CUDA graph, so a
  * run of the whole group is one graph launch.  A member whose energy program
  * alone exceeds pass_budget with its chain states cached takes the recompute
- * form (program choice bit 5) when that fits.  TN_ERR_OVER_BUDGET when a
+ * form (program choice bit 5) when that fits, in FP64 and FP32 else the
+ * products without digit planes (bit 3 cleared: the same values to rounding),
+ * else both; where the shared arena exceeds the remaining budget, every FP64
+ * and FP32 member goes without digit planes.  TN_ERR_OVER_BUDGET when a
  * member alone still exceeds pass_budget or the arena the remaining budget;
  * TN_ERR_NO_DEVICE without a device.  Inputs and results are concatenated in
  * member order with the layouts of tn_batch_*; member k of the generator
@@ -310,8 +316,10 @@ typedef struct {
 
 /* Queue a job.  It is admitted to the GPU when its exact footprint fits the
  * budget left by running jobs; jobs that can never fit return
- * TN_ERR_OVER_BUDGET here.  Jobs take the tuning table's program choices and
- * do not fall back to the recompute form: a job whose cached-state program
+ * TN_ERR_OVER_BUDGET here.  Jobs take the tuning table's program choices; an
+ * FP64 or FP32 job over the whole budget takes the products without digit
+ * planes (bit 3 cleared: the same values to rounding) if that fits.  They do
+ * not fall back to the recompute form: a job whose cached-state program
  * exceeds the budget would hold the device for seconds to minutes, which a
  * latency-bound stream refuses instead (set bit 5 for the shape by hand to
  * serve it).  Admitted jobs run concurrently with earlier ones:
@@ -453,13 +461,15 @@ tn_status tn_ite_run(tn_lattice *lat, const tn_ite_params *params, double *energ
  * 15 (bits 0-3 set) is the fixed default; codes run from 0 to 63.  tn_autotune times every combination that
  * changes the program of each distinct (L[k], W[k], D[k]) on a batch of
  * copies of it (as many as fit max_bytes, 0 = 4 GiB, at most 64; shapes whose
- * single footprint exceeds max_bytes are skipped), `reps` timed runs after one
+ * single footprint exceeds max_bytes are skipped; where only the digit planes
+ * of bit 3 make it too large for max_bytes or the budget left, the choices are
+ * timed without them), `reps` timed runs after one
  * warm-up, CUDA events on the batch's stream, and stores the fastest (a
  * combination replaces the current choice only when 2% faster) in a process-
  * wide table keyed on (L, W, D, precision, work).  Batches, lattices and served
  * jobs created afterwards use the table's choice for their shape, so a lattice
- * is contracted the same way alone, in a batch and when served; tune before
- * creating them.  work: TN_WORK_NORM or TN_WORK_ENERGY. */
+ * is contracted the same way alone, in a batch and when served as long as the
+ * budget left holds that choice (tn_energy); tune before creating them.  work: TN_WORK_NORM or TN_WORK_ENERGY. */
 tn_status tn_autotune(tn_ctx *ctx, int n, const int *L, const int *W, const int *D, tn_precision prec,
                       tn_work work, int reps, size_t max_bytes);
 /* The table's choice for a shape: knobs (15 if untuned), the tuned and the

@@ -5,6 +5,7 @@
 // the table's choice for its shape, so a lattice is contracted the same way
 // (and gives the same bits) alone, in any batch and when served.  The knobs
 // are all exact reformulations; only speed differs.
+#include <algorithm>
 #include <cstdio>
 #include <map>
 #include <mutex>
@@ -92,11 +93,25 @@ tn_status tn_autotune(tn_ctx* ctx, int n, const int* L, const int* W, const int*
         tn_status result = TN_OK;
         for (const auto& sh : shapes) {
             const int l = std::get<0>(sh.first), w = std::get<1>(sh.first), d = std::get<2>(sh.first);
-            // copies of the shape filling at most max_bytes (between 1 and 64)
-            tn_batch* probe = nullptr;
+            // copies of the shape filling at most max_bytes (between 1 and 64).  Where not even one
+            // fits with digit planes, the choices are timed without them, as calls will run there
+            auto footprint = [&](int code, size_t* bytes) {
+                tn_batch* probe = nullptr;
+                BatchOpts o;
+                o.knobs = code;
+                const tn_status s = batch_create(ctx, 1, &l, &w, &d, prec, TN_SCHED_AUTO, work, false, &probe, bytes, &o);
+                if (probe) batch_destroy(probe);
+                return s;
+            };
             size_t fp = 0;
-            tn_status st = batch_create(ctx, 1, &l, &w, &d, prec, TN_SCHED_AUTO, work, false, &probe, &fp);
-            if (probe) batch_destroy(probe);
+            tn_status st = footprint(tuned_knobs(l, w, d, prec, work).code(), &fp);
+            const size_t used = ctx->used.load(), left = ctx->budget > used ? ctx->budget - used : 0;
+            int drop = 0;
+            if (st == TN_OK && fp > std::min(max_bytes, left) && (prec == TN_FP64 || prec == TN_FP32)) {
+                size_t f2 = 0;
+                st = footprint(kDefaultKnobs & ~kTensorKnob, &f2);
+                if (st == TN_OK && f2 <= std::min(max_bytes, left)) { fp = f2; drop = kTensorKnob; }
+            }
             if (st != TN_OK) { result = st; break; }
             if (fp > max_bytes) continue;                 // too large to tune within the limit
             const int copies = (int)std::max<size_t>(1, std::min<size_t>(64, max_bytes / std::max<size_t>(fp, 1)));
@@ -109,7 +124,7 @@ tn_status tn_autotune(tn_ctx* ctx, int n, const int* L, const int* W, const int*
             double best_ms = -1.0;
             for (int code : cands) {
                 BatchOpts opts;
-                opts.knobs = code;
+                opts.knobs = code & ~drop;
                 tn_batch* b = nullptr;
                 st = batch_create(ctx, copies, Ls.data(), Ws.data(), Ds.data(), prec, TN_SCHED_AUTO, work, true, &b,
                                   nullptr, &opts);
