@@ -103,24 +103,23 @@ __device__ inline void block_jacobi(T* A, int m, int n, long long lda, T* V, lon
 // one dot product, not three.  The ITE's FP64 updates take it (4 steps of 6x6
 // D=2: 11.1 -> 9.0 ms).  The FP32 boundary MPS does not: its ill-conditioned
 // states turn any change of rounding into 1e-4 of an observable.
-template <typename T>
-__device__ inline void block_jacobi_carried(T* A, int m, int n, long long lda, T* V, long long ldv, int* flag) {
-    const T tol = sizeof(T) == 8 ? T(1e-15) : T(1e-6);
+__device__ inline void block_jacobi_carried(double* A, int m, int n, long long lda, double* V, long long ldv,
+                                            int* flag) {
+    constexpr double tol = 1e-15;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
     const int n2 = n + (n & 1);
-    __shared__ T fro_part[32];
-    __shared__ T nrm[kJacobiMaxCols];
-    if (V)
-        for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
-            const int c = idx / n, r = idx - c * n;
-            V[c * ldv + r] = r == c ? T(1) : T(0);
-        }
-    T negligible = 0;
+    __shared__ double fro_part[32];
+    __shared__ double nrm[kJacobiMaxCols];
+    for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
+        const int c = idx / n, r = idx - c * n;
+        V[c * ldv + r] = r == c ? 1.0 : 0.0;
+    }
+    double negligible = 0;
     for (int sweep = 0; sweep < kJacobiMaxSweeps && n > 1; ++sweep) {
-        T f2 = 0;
+        double f2 = 0;
         for (int c = warp; c < n; c += nwarps) {
-            const T* ca = A + c * lda;
-            T s = 0;
+            const double* ca = A + c * lda;
+            double s = 0;
             for (int r = lane; r < m; r += 32) s += ca[r] * ca[r];
             s = jacobi_warp_sum(s);
             if (lane == 0) nrm[c] = s;
@@ -129,7 +128,7 @@ __device__ inline void block_jacobi_carried(T* A, int m, int n, long long lda, T
         if (sweep == 0) {
             if (lane == 0) fro_part[warp] = f2;
             __syncthreads();
-            T fro2 = 0;
+            double fro2 = 0;
             for (int w = 0; w < nwarps; ++w) fro2 += fro_part[w];
             negligible = tol * tol * fro2;
         }
@@ -145,35 +144,33 @@ __device__ inline void block_jacobi_carried(T* A, int m, int n, long long lda, T
                 }
                 if (a > b) { const int t = a; a = b; b = t; }
                 if (b >= n) continue;              // the padding column is zero
-                const T al = nrm[a], be = nrm[b];
+                const double al = nrm[a], be = nrm[b];
                 if (!(al > negligible) || !(be > negligible)) continue;
-                T* ca = A + a * lda;
-                T* cb = A + b * lda;
-                T ga = 0;
+                double* ca = A + a * lda;
+                double* cb = A + b * lda;
+                double ga = 0;
                 for (int r = lane; r < m; r += 32) ga += ca[r] * cb[r];
                 ga = jacobi_warp_sum(ga);
-                if (ga == T(0) || fabs(ga) <= tol * sqrt(al * be)) continue;
-                const T zeta = (be - al) / (T(2) * ga);
-                const T t = (zeta >= T(0) ? T(1) : T(-1)) / (fabs(zeta) + sqrt(T(1) + zeta * zeta));
-                const T c = T(1) / sqrt(T(1) + t * t), s = c * t;
+                if (ga == 0.0 || fabs(ga) <= tol * sqrt(al * be)) continue;
+                const double zeta = (be - al) / (2.0 * ga);
+                const double t = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
+                const double c = 1.0 / sqrt(1.0 + t * t), s = c * t;
                 if (lane == 0) {
                     *flag = 0;
                     nrm[a] = al - t * ga;
                     nrm[b] = be + t * ga;
                 }
                 for (int r = lane; r < m; r += 32) {
-                    const T x = ca[r], y = cb[r];
+                    const double x = ca[r], y = cb[r];
                     ca[r] = c * x - s * y;
                     cb[r] = s * x + c * y;
                 }
-                if (V) {
-                    T* va = V + a * ldv;
-                    T* vb = V + b * ldv;
-                    for (int r = lane; r < n; r += 32) {
-                        const T x = va[r], y = vb[r];
-                        va[r] = c * x - s * y;
-                        vb[r] = s * x + c * y;
-                    }
+                double* va = V + a * ldv;
+                double* vb = V + b * ldv;
+                for (int r = lane; r < n; r += 32) {
+                    const double x = va[r], y = vb[r];
+                    va[r] = c * x - s * y;
+                    vb[r] = s * x + c * y;
                 }
                 __syncwarp();
             }
