@@ -447,6 +447,7 @@ void materialize(tn_batch* b, char* base, std::vector<char>* tasks_out, std::vec
             P.level = L.level;
             P.dt = b->dt;
             P.variant = vr.first;
+            P.rest = true;
             P.ntasks = (int)vr.second.size();
             align_group();
             P.task_off = tasks.size();
@@ -718,7 +719,7 @@ cudaError_t issue(tn_batch* b, cudaStream_t st, std::vector<std::pair<cudaEvent_
             case OP_GEMM:
             case OP_GEMM_DOT:
                 e = launch_gemm(L.dt, L.kind == OP_GEMM_DOT, static_cast<const GemmTask*>(tp), L.ntasks,
-                                L.nblocks, slots, st, L.variant);
+                                L.nblocks, slots, st, L.variant, L.rest);
                 break;
             case OP_ABSORB2:
             case OP_ABSORB2_DOT:

@@ -39,6 +39,7 @@ struct Launch {
     int ntasks = 0;
     long long nblocks = 0;
     double bytes = 0, macs = 0;
+    bool rest = false;    // products: only what the digits left (launch_gemm)
 };
 
 struct Member {

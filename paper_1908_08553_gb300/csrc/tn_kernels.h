@@ -225,8 +225,9 @@ cudaError_t launch_absorb2(bool dot, int K1, int N2, const AbsorbTask* tasks, in
                            Slot* slots, cudaStream_t st, const int* tmap = nullptr, int rev = 0);
 // variant 0: 64x64 tiles, any dtype; 1: FP32 128x128 double-buffered with
 // 16-byte loads; 2: the same with scalar loads (odd extents, e.g. D = 3).
+// rest: the outputs that products from digits left to the pipe (GemmTask::flags).
 cudaError_t launch_gemm(int dt, bool dot, const GemmTask* tasks, int ntasks, long long nblocks,
-                        Slot* slots, cudaStream_t st, int variant = 0);
+                        Slot* slots, cudaStream_t st, int variant = 0, bool rest = false);
 int gemm_variant(int dt, long long M, long long N, long long K, long long sam, long long sak, long long sbk,
                  long long sbn);
 long long gemm_tiles_v(int variant, long long M, long long N, int* tiles_n);
