@@ -138,7 +138,7 @@ void materialize(tn_batch* b, char* base, std::vector<char>* tasks_out, std::vec
     // FP64 in 16 x 16 tiles: a few flagged ones spread over the SMs (128 x 128 of them on
     // one SM would take 2 x 128 x 128 / 4 = 8192 cycles a term)
     auto pipe_variant = [&](const Op& op) {
-        return b->dt == 0 ? kGemmSmall : gemm_variant(b->dt, op.gm, op.gn, op.gk, op.sam, op.sak, op.sbk, op.sbn);
+        return b->dt == 0 ? kGemmSmallRest : gemm_variant(b->dt, op.gm, op.gn, op.gk, op.sam, op.sak, op.sbk, op.sbn);
     };
     // partial region placement needs npart first: count dot tiles
     for (auto& kv : groups) {
@@ -451,15 +451,26 @@ void materialize(tn_batch* b, char* base, std::vector<char>* tasks_out, std::vec
             P.ntasks = (int)vr.second.size();
             align_group();
             P.task_off = tasks.size();
-            long long tile0 = 0;
+            // FP64: 1 or 8 such tiles a block, with the same partial sums.  Mostly none is flagged
+            // and 3 ns a block is all there is: of the 4.3 ms of 256 8x8 D=2 energies (77.3 ms)
+            // 0.8 are left with 8.  In launches of few tiles 8 would leave SMs idle where some
+            // are flagged (a frustrated seam, 8x8 D=2 1.6 against 2.5 ms, 10x10 33.6 against 38.9)
+            long long tiles = 0, tile0 = 0;
+            int tn_;
+            for (const OpRef& r : vr.second) {
+                const Op& op = b->m[r.member].pg->ops[r.op];
+                tiles += gemm_tiles_v(vr.first, op.gm, op.gn, &tn_);
+            }
+            const int per = b->dt == 0 && tiles > 49152 ? 8 : 1;
             for (const OpRef& r : vr.second) {
                 const Op& op = b->m[r.member].pg->ops[r.op];
                 GemmTask t = gemm_task(r, op.A_src, op.B_src, kind == OP_TC_GEMM_DOT, vr.first, tile0);
+                if (b->dt == 0) t.ksplit = per;
                 t.flags = static_cast<const unsigned long long*>(tensor_ptr(r.member, op.adj));
                 t.flags_n = (int)((op.gn + 127) / 128);
                 t.slot_flags = slot_of(r.member, op.adj);
                 append(&t, sizeof(t));
-                tile0 += t.ntiles;
+                tile0 += t.ntiles / per;
             }
             P.nblocks = tile0;
             b->launches.push_back(P);

@@ -60,7 +60,7 @@ struct GemmTask {
     long long tile0;
     long long kslice;     // k per tile (= K unless the product is split along k)
     int tiles_n, ntiles;
-    int ksplit;           // tiles along k (dot mode: one FP64 partial each)
+    int ksplit;           // tiles along k (dot mode: one FP64 partial each); kGemmSmallRest: tiles per block
     int slot_A, slot_B, slot_C, slot_D;
     // after a product from digits (else null): only the tiles its guard names
     // (SliceGuardTask::flags), their dot added to the slot's
@@ -336,6 +336,7 @@ cudaError_t launch_absorb_dot_plain(int dt, const void* in, const void* E, const
 constexpr int kAbsorbThreads = 256;
 constexpr int kGemmTile = 64;
 constexpr int kGemmSmall = 7;             // variant of the FP64 products of few outputs
+constexpr int kGemmSmallRest = 8;         // ... and of the outputs FP64 products from digits leave
 constexpr int kDotPerBlock = 4096;
 long long absorb_tiles(long long P, long long S, int K, int N);
 bool absorb_has_fast_path(int K, int N);
