@@ -184,3 +184,32 @@ def test_fp32_products_of_small_rows_and_columns(ctx):
     for knobs in (NO_PLANES, 15):
         norm, _, _, _ = _full(ctx, L, W, D, A, knobs, tn.TN_FP32)
         assert _off(norm, ref) <= 2e-5, knobs
+
+
+# outputs left to the pipe in a large launch (8 of its 16 x 16 tiles a block) and in a
+# small one (one a block): the same sums in the same order, so the same bits.  256^3 and
+# 729^3 products (ragged last tiles of a row); the batches' launches have more than
+# 49,152 tiles, those of one lattice fewer.
+@pytest.mark.parametrize("L,W,D,n", [(8, 8, 2, 128), (6, 6, 3, 24)])
+def test_batches_of_graded_states_equal_alone(ctx, L, W, D, n):
+    kinds = [parity_state(L, W, 2.0 ** -20, 4600, D), inputs.random_lattice(L, W, D, 4601),
+             parity_state(L, W, 2.0 ** -12, 4602, D)]
+    if D == 2:
+        kinds.append(seam_ising(L, W, 1.5))
+    b, rows = tn.tn_batch_create(ctx, [L] * n, [W] * n, [D] * n, tn.TN_FP64), []
+    try:
+        tn.tn_batch_set_tensors(b, np.concatenate([kinds[k % len(kinds)] for k in range(n)]))
+        tn.tn_batch_run(b, 1.0, np.full(n, 3.04))
+        got = tn.tn_batch_results_host(b).reshape(n, -1)
+    finally:
+        tn.tn_batch_destroy(b)
+    for A in kinds:
+        b1 = tn.tn_batch_create(ctx, [L], [W], [D], tn.TN_FP64)
+        try:
+            tn.tn_batch_set_tensors(b1, A)
+            tn.tn_batch_run(b1, 1.0, np.full(1, 3.04))
+            rows.append(tn.tn_batch_results_host(b1).copy())
+        finally:
+            tn.tn_batch_destroy(b1)
+    for k in range(n):
+        assert np.array_equal(got[k], rows[k % len(kinds)]), k
